@@ -70,14 +70,18 @@ struct BatchGeo {
 
 // MIXED selects the mixed-precision body (wcns_mixed_body.cuh).  Mixed
 // tiles target BATCH_MIXED_WARPS resident warps per SM (a register cap of
-// 65536 / (32 BATCH_MIXED_WARPS) per thread); the FP64 body keeps its
-// registers.  On the 4096-problem batch 32 warps (64 registers, more
+// 65536 / (32 BATCH_MIXED_WARPS) per thread), FP64 tiles BATCH_FP64_WARPS
+// (4096 problems: 8 / 12 / 16 / 20 warps 23.3 / 21.6 / 21.5 / 21.9 ms a
+// step).  On the 4096-problem batch 32 warps (64 registers, more
 // spills) beat 28, 24, 20 and 16: the single-pass body is latency bound.
+#ifndef BATCH_FP64_WARPS
+#define BATCH_FP64_WARPS 16
+#endif
 #ifndef BATCH_MIXED_WARPS
 #define BATCH_MIXED_WARPS 32
 #endif
 template <bool MIXED, class T>
-__global__ void __launch_bounds__(T::THREADS, MIXED ? BATCH_MIXED_WARPS * 32 / T::THREADS : 1)
+__global__ void __launch_bounds__(T::THREADS, MIXED ? BATCH_MIXED_WARPS * 32 / T::THREADS : BATCH_FP64_WARPS * 32 / T::THREADS)
     batch_sweep_kernel(const SweepArgs a, const BatchArgs b) {
   extern __shared__ double smem_raw[];
   for (int t = blockIdx.x; t < b.ntiles; t += gridDim.x) {
@@ -209,7 +213,7 @@ struct Batch2Geo {
 // One direction of one stage of every problem: a persistent loop over the
 // direction's work list.
 template <bool MIXED, int DIR, class T>
-__global__ void __launch_bounds__(T::THREADS, MIXED ? 3 : 1)
+__global__ void __launch_bounds__(T::THREADS, MIXED ? 3 : BATCH_FP64_WARPS * 32 / T::THREADS)
     batch2_sweep_kernel(const SweepArgs a, const Batch2Args b) {
   extern __shared__ double smem_raw[];
   for (int t = blockIdx.x; t < b.ntiles; t += gridDim.x) {

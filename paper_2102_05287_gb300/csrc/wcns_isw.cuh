@@ -1,0 +1,354 @@
+// WCNS-IS interpolation (Sec. 4.3) of FP64 deviations without FP64
+// arithmetic.
+//
+// Why: an FP64 warp instruction occupies an SM's FP64 units for 16 cycles on
+// GB300, an FP32 or integer one its 128 lanes for a quarter to half a cycle,
+// and the interpolation's ~65 operations a value were 70 % of the FP64
+// sweeps' FP64 work (1034 to 1110 add/mul/fma per cell and direction before,
+// about 380 after: 27.4 against 11.0 ms a step of the 2048 x 1024
+// shock/bubble run, 43.6 against 22.2 ms of a 120^3 bubble collapse).
+//
+// How: the interpolated value is the linear fifth-order one plus a correction
+// by the nonlinear weights,
+//   u = u_lin + sum_k d_k rho_k (s_k - u_lin) / (1 + sum_k d_k rho_k),
+//   rho_0 = tau^2 / (b0 b01), rho_1 = tau^2 / (b1 b01), rho_{2,3} = tau / b_{2,3}
+// (d_k the linear weights, b_k = beta_k + eps, s_k the sub-stencil values).
+// - The five deviations become integers on a common binary scale, so that
+//   u_lin, s_k - u_lin and every difference in the indicators are exact.
+// - The correction is formed in FP32, relative error below 2^-19, and where
+//   that is not enough in pairs of FP32 values, below 2^-39; both errors are
+//   bounded by S = sum d_k rho_k |s_k - u_lin| / (1 + sum d_k rho_k).
+// - A value is accepted where the bound is at most 2^-54 (scale + |u|), a
+//   quarter of the rounding of the sum scale + u that the caller forms.
+//   Elsewhere (strong jumps of the field inside the stencil) the caller
+//   evaluates the printed formula in FP64.
+// Every decision depends on the value's own stencil only.
+#pragma once
+#include <math.h>
+#include <stdint.h>
+#include <string.h>
+
+#ifdef __CUDACC__
+#define WISW __host__ __device__ __forceinline__
+#else
+#define WISW static inline
+#endif
+
+namespace wcns {
+namespace isw {
+
+// --- bit-level helpers (device intrinsics; plain C++ on the host) ----------
+WISW unsigned hi32(double x) {
+#ifdef __CUDA_ARCH__
+  return (unsigned)__double2hiint(x);
+#else
+  uint64_t u;
+  memcpy(&u, &x, 8);
+  return (unsigned)(u >> 32);
+#endif
+}
+WISW unsigned lo32(double x) {
+#ifdef __CUDA_ARCH__
+  return (unsigned)__double2loint(x);
+#else
+  uint64_t u;
+  memcpy(&u, &x, 8);
+  return (unsigned)u;
+#endif
+}
+WISW double from_bits(uint64_t u) {
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)u);
+#else
+  double x;
+  memcpy(&x, &u, 8);
+  return x;
+#endif
+}
+WISW float from_bits32(unsigned u) {
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(u);
+#else
+  float x;
+  memcpy(&x, &u, 4);
+  return x;
+#endif
+}
+WISW int clz32(unsigned u) {
+#ifdef __CUDA_ARCH__
+  return __clz((int)u);
+#else
+  return u ? __builtin_clz(u) : 32;
+#endif
+}
+WISW float fdiv(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fdividef(a, b);
+#else
+  return a / b;
+#endif
+}
+WISW float frcp(float b) {
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+  return r;
+#else
+  return 1.0f / b;
+#endif
+}
+WISW float frsqrt(float b) {
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+  return r;
+#else
+  return 1.0f / sqrtf(b);
+#endif
+}
+WISW int frint(float x) {
+#ifdef __CUDA_ARCH__
+  return __float2int_rn(x);
+#else
+  return (int)nearbyintf(x);
+#endif
+}
+
+// --- fixed point -----------------------------------------------------------
+// x as an integer multiple of 2^-54 of the binade top above exponent field
+// E (|x| < 2^(E - 1022)), truncated toward zero: |fix| < 2^54.  Zeros and
+// subnormals give 0.
+WISW int64_t fix(double x, int E) {
+  const unsigned h = hi32(x), l = lo32(x);
+  const int e = (int)((h >> 20) & 0x7FFu);
+  const unsigned m = (h & 0xFFFFFu) | 0x100000u;
+  const uint64_t f = ((((uint64_t)m << 32) | l) << 1);
+  const int s = E - e;
+  const int64_t v = (s < 64 && e != 0) ? (int64_t)(f >> s) : 0;
+  return (int)h < 0 ? -v : v;
+}
+// v 2^(E - 1022 - 61) rounded to nearest FP64 (|v| < 2^63, 64 <= E <= 2040).
+WISW double unfix(int64_t v, int E) {
+  if (v == 0) return 0.0;
+  const uint64_t sgn = (uint64_t)(v >> 63);
+  uint64_t a = ((uint64_t)v ^ sgn) - sgn;
+  const unsigned ah = (unsigned)(a >> 32);
+  const int n = ah ? clz32(ah) : 32 + clz32((unsigned)a);
+  a <<= n;  // leading bit at 2^63
+  const uint64_t m = (a >> 11) + ((a >> 10) & 1u);
+  return from_bits((sgn << 63) + ((uint64_t)(unsigned)(E + 2 - n) << 52) + m);
+}
+// v / 2^32 in FP32, relative error below 2^-23 plus 2^-24 absolute
+// (|v| <= 2^56)
+WISW float fx(int64_t v) {
+  return fmaf((float)((unsigned)v >> 8), 5.9604644775390625e-08f, (float)(int)(v >> 32));
+}
+
+// --- FP32 pairs ------------------------------------------------------------
+struct F2 {
+  float h, l;
+};
+WISW F2 fx2(int64_t v) {
+  const float a = (float)(int)(v >> 32), b = (float)((unsigned)v >> 8) * 5.9604644775390625e-08f;
+  const float s = a + b;
+  return {s, b - (s - a)};
+}
+WISW F2 mul(F2 a, F2 b) {
+  const float p = a.h * b.h;
+  float e = fmaf(a.h, b.h, -p);
+  e = fmaf(a.h, b.l, e);
+  e = fmaf(a.l, b.h, e);
+  return {p, e};
+}
+WISW F2 sqr(F2 a) {
+  const float p = a.h * a.h;
+  return {p, fmaf(a.h + a.h, a.l, fmaf(a.h, a.h, -p))};
+}
+WISW F2 scale(F2 a, float s) { return {a.h * s, a.l * s}; }  // s a power of two
+WISW F2 add(F2 a, F2 b) {
+  const float s = a.h + b.h, t = s - a.h;
+  const float e = (a.h - (s - t)) + (b.h - t);
+  return {s, e + (a.l + b.l)};
+}
+// a / b
+WISW F2 div(F2 a, F2 b) {
+  const float r = frcp(b.h), q = a.h * r;
+  const float d = fmaf(-q, b.l, fmaf(-q, b.h, a.h) + a.l);
+  return {q, d * r};
+}
+
+// One side's stencil in integers: the differences around the upwind node.
+//   d0 = u_{i+1} - u_i, dm the difference on the far side of the upwind node,
+//   Da, Db, Dc second differences at the node behind the upwind node, at it,
+//   and at the downwind one; c* the first-difference parts of the indicators.
+struct Side {
+  int64_t dm, Da, Db, Dc, c01, c2, c3;
+};
+
+constexpr float K133 = 13.0f / 3.0f;
+constexpr float K133L = (float)(13.0 / 3.0 - (double)K133);
+constexpr float UNIT = 4194304.0f;  // 2^22: the FP32 image of the largest |U|
+constexpr float FLOORB = 256.0f;    // 2^-36 UNIT^2: smallest indicator taken as is
+
+struct E4 {
+  int64_t e0, e1, e2, e3;  // 128 (s_k - u_lin)
+};
+WISW E4 offsets(const Side &s) {
+  const int64_t m = 3 * s.Da;
+  E4 e;
+  e.e0 = 5 * s.Dc - m + (s.Db << 4) - (s.Db << 1);
+  e.e1 = e.e0 - (s.Db << 6);
+  e.e2 = e.e0 - (s.Dc << 4);
+  e.e3 = e.e1 + (m << 4);
+  return e;
+}
+
+// FP32 evaluation: the weighted correction 128 (u - u_lin) in units of 2^39,
+// and the bounds' ingredients.
+struct Est {
+  float corr, S, G, minb, mint, flr;
+};
+WISW Est side32(const Side &s, const E4 &e, float d0, float eps) {
+  const float dm = fx(s.dm), Da = fx(s.Da), Db = fx(s.Db), Dc = fx(s.Dc);
+  const float c01 = fx(s.c01), c2 = fx(s.c2 >> 2), c3 = fx(s.c3 >> 2);
+  const float ta = fx((s.Da - 2 * s.Db + s.Dc) >> 2), tc = fx((s.Da - s.Dc) >> 2);
+  const float b0 = fmaf(4.0f * d0, d0, eps), b1 = fmaf(4.0f * dm, dm, eps);
+  const float b01 = fmaf(K133 * Db, Db, fmaf(c01, c01, eps));
+  const float b2 = fmaf(K133 * Dc, Dc, fmaf(16.0f * c2, c2, eps));
+  const float b3 = fmaf(K133 * Da, Da, fmaf(16.0f * c3, c3, eps));
+  const float tau = 16.0f * fmaf(K133 * ta, ta, tc * tc);
+  Est r;
+  r.minb = fminf(fminf(fminf(b0, b1), fminf(b2, b3)), b01);
+  r.mint = fminf(r.minb, fmaxf(tau, 1.4551915228366852e-11f));  // 2^-36
+  r.flr = 0.0f;
+  if (r.minb < FLOORB) {
+    // Indicators below FLOORB: taken as FLOORB.  Where they are exact zeros,
+    // and every other indicator and tau at least 2^16 FLOORB, their
+    // sub-stencils carry the result up to 2^-14 either way.
+    const float big = 65536.0f * FLOORB;
+    const auto fine = [&](float b) { return b <= eps || b >= big; };
+    r.flr = fine(b0) && fine(b1) && fine(b01) && fine(b2) && fine(b3) && (tau >= big || tau == 0.0f)
+                ? 9.765625e-4f * UNIT : 16.0f * UNIT;
+  }
+  const float r01 = fdiv(tau, fmaxf(b01, FLOORB));
+  const float w0 = 15.0f * fdiv(tau, fmaxf(b0, FLOORB)) * r01;
+  const float w1 = 5.0f * fdiv(tau, fmaxf(b1, FLOORB)) * r01;
+  const float w2 = 10.0f * fdiv(tau, fmaxf(b2, FLOORB));
+  const float w3 = 2.0f * fdiv(tau, fmaxf(b3, FLOORB));
+  const float g = (w0 + w1) + (w2 + w3);
+  const float inv = frcp(32.0f + g);
+  const float a0 = w0 * fx(e.e0 >> 7), a1 = w1 * fx(e.e1 >> 7), a2 = w2 * fx(e.e2 >> 7), a3 = w3 * fx(e.e3 >> 7);
+  r.corr = ((a0 + a1) + (a2 + a3)) * inv;
+  r.S = ((fabsf(a0) + fabsf(a1)) + (fabsf(a2) + fabsf(a3))) * inv;
+  r.G = g * inv;
+  return r;
+}
+
+// The same correction in FP32 pairs.  kd: (13/3) D^2 of the two shared
+// second differences, kDb at Db, kDc at Dc; b0: 4 d0^2.
+WISW F2 side2(const Side &s, const E4 &e, F2 b0, F2 kDb, F2 kDc, F2 eps, bool use_eps) {
+  const F2 K = {K133, K133L};
+  F2 b1 = scale(sqr(fx2(s.dm)), 4.0f);
+  F2 b01 = add(sqr(fx2(s.c01)), kDb);
+  F2 b2 = add(scale(sqr(fx2(s.c2 >> 2)), 16.0f), kDc);
+  F2 b3 = add(scale(sqr(fx2(s.c3 >> 2)), 16.0f), mul(K, sqr(fx2(s.Da))));
+  const F2 tau = scale(add(mul(K, sqr(fx2((s.Da - 2 * s.Db + s.Dc) >> 2))), sqr(fx2((s.Da - s.Dc) >> 2))), 16.0f);
+  if (use_eps) {
+    b0 = add(b0, eps);
+    b1 = add(b1, eps);
+    b01 = add(b01, eps);
+    b2 = add(b2, eps);
+    b3 = add(b3, eps);
+  }
+  const F2 r01 = div(tau, b01);
+  F2 w0 = mul(div(tau, b0), r01), w1 = mul(div(tau, b1), r01), w2 = div(tau, b2), w3 = div(tau, b3);
+  // 15, 5, 10, 2 times: exact in the pair up to the rounding of the products
+  w0 = mul(w0, {15.0f, 0.0f});
+  w1 = mul(w1, {5.0f, 0.0f});
+  w2 = mul(w2, {10.0f, 0.0f});
+  w3 = scale(w3, 2.0f);
+  const F2 den = add(add(add(w0, w1), add(w2, w3)), {32.0f, 0.0f});
+  const F2 num = add(add(mul(w0, fx2(e.e0 >> 7)), mul(w1, fx2(e.e1 >> 7))),
+                     add(mul(w2, fx2(e.e2 >> 7)), mul(w3, fx2(e.e3 >> 7))));
+  return div(num, den);
+}
+
+// c (in units of 2^39) as an integer
+WISW int64_t corr_int(F2 c) {
+  const int i1 = frint(c.h);
+  const float f = c.h - (float)i1;
+  const int i2 = frint(f * 2147483648.0f * 0.5f), i3 = frint(c.l * 2147483648.0f * 0.5f);
+  return ((int64_t)i1 << 39) + (((int64_t)i2 + (int64_t)i3) << 9);
+}
+
+// WCNS-IS of the deviations um2, um1, (0), up1, up2, up3 of nodes i-2 .. i+3
+// from node i: left-biased value ul and right-biased value ur at i+1/2.
+// e4: 4 eps.  scale: the magnitude whose rounding the result may carry.
+// Bit 0 / 1 set: ul / ur is within 2^-54 (scale + |u|) of the exact value
+// plus the fixed-point rounding; clear: not decided.  bit 2: pairs used.
+WISW int interpolate(double um2, double um1, double up1, double up2, double up3, double e4, float scl, double &ul,
+                     double &ur) {
+  unsigned mx = hi32(um2) & 0x7FFFFFFFu, t;
+  t = hi32(um1) & 0x7FFFFFFFu;
+  mx = t > mx ? t : mx;
+  t = hi32(up1) & 0x7FFFFFFFu;
+  mx = t > mx ? t : mx;
+  t = hi32(up2) & 0x7FFFFFFFu;
+  mx = t > mx ? t : mx;
+  t = hi32(up3) & 0x7FFFFFFFu;
+  mx = t > mx ? t : mx;
+  const int E = (int)(mx >> 20);
+  ul = ur = 0.0;
+  if (E < 64 || E > 2040) return mx == 0 ? 3 : 0;  // zeros; or outside the range below
+  const int64_t X0 = fix(um2, E), X1 = fix(um1, E), X3 = fix(up1, E), X4 = fix(up2, E), X5 = fix(up3, E);
+  const int64_t dm2 = X1 - X0, dm1 = -X1, d1 = X4 - X3, d2 = X5 - X4;
+  const int64_t Dm = dm1 - dm2, D0 = X3 - dm1, D1 = d1 - X3, D2 = d2 - d1;
+  const Side L = {dm1, Dm, D0, D1, dm1 + X3, 3 * X3 - d1, 3 * dm1 - dm2};
+  const Side R = {d1, D2, D1, D0, X3 + d1, 3 * X3 - dm1, 3 * d1 - d2};
+  const E4 eL = offsets(L), eR = offsets(R);
+  // 4 eps in units of (2^(E-1022) / 2^22)^2 and the scale in units of
+  // 2^(E-1022) / 2^22, exponents clamped to FP32's range (a larger eps
+  // only lowers the already negligible weights; a smaller scale is safe)
+  const unsigned eh = hi32(e4);
+  int ee = (int)(eh >> 20) - 1023 - 2 * (E - 1022) + 44;
+  ee = ee > 100 ? 100 : ee;
+  const float eps = ee < -100 ? 0.0f : from_bits32(((unsigned)(ee + 127) << 23) | ((eh & 0xFFFFFu) << 3) | (lo32(e4) >> 29));
+  int es = 1022 - E + 22;
+  es = es > 100 ? 100 : (es < -120 ? -120 : es);
+  const float sc = scl * from_bits32((unsigned)(es + 127) << 23);
+  const float fd0 = fx(X3);
+  const Est a = side32(L, eL, fd0, eps), b = side32(R, eR, fd0, eps);
+  const float linL = fx(((X3 << 6) - eL.e0) >> 7), linR = fx(((X3 << 6) - eR.e0) >> 7);
+  // what the result may be off by: 2^-54 (scale + |u|)
+  const float tolL = 5.551115123125783e-17f * (sc + fabsf(linL + a.corr));
+  const float tolR = 5.551115123125783e-17f * (sc + fabsf(linR + b.corr));
+  const float mtol = 2.3283064365386963e-10f;  // 2^-54 UNIT
+  const float xL = 1.9073486328125e-06f * frsqrt(a.mint), xR = 1.9073486328125e-06f * frsqrt(b.mint);  // 2^-19 /
+  const bool baseL = tolL >= mtol, baseR = tolR >= mtol;
+  const bool okL = baseL && a.S * (1.9073486328125e-06f + xL) + a.flr <= tolL;
+  const bool okR = baseR && b.S * (1.9073486328125e-06f + xR) + b.flr <= tolR;
+  F2 cL = {a.corr, 0.0f}, cR = {b.corr, 0.0f};
+  int ret = (okL ? 1 : 0) | (okR ? 2 : 0);
+  if (ret != 3) {
+    const bool goL = !okL && baseL && a.minb >= FLOORB &&
+                     a.S * (4.547473508864641e-13f + xL) + 2.384185791015625e-07f * a.G <= tolL;
+    const bool goR = !okR && baseR && b.minb >= FLOORB &&
+                     b.S * (4.547473508864641e-13f + xR) + 2.384185791015625e-07f * b.G <= tolR;
+    if (goL || goR) {
+      const F2 K = {K133, K133L};
+      const F2 k0 = mul(K, sqr(fx2(D0))), k1 = mul(K, sqr(fx2(D1)));
+      const F2 b0 = isw::scale(sqr(fx2(X3)), 4.0f);
+      const F2 ep = {eps, eps == 0.0f ? 0.0f : from_bits32((unsigned)(ee + 127) << 23) * ((float)(lo32(e4) & 0x1FFFFFFFu) * 2.220446049250313e-16f)};
+      const float neg = 7.0368744e13f * eps;  // 2^46 eps
+      if (goL) cL = side2(L, eL, b0, k0, k1, ep, a.minb < neg);
+      if (goR) cR = side2(R, eR, b0, k1, k0, ep, b.minb < neg);
+      ret |= (goL ? 5 : 0) | (goR ? 6 : 0);
+    }
+  }
+  ul = unfix((X3 << 6) - eL.e0 + corr_int(cL), E);
+  ur = unfix((X3 << 6) - eR.e0 + corr_int(cR), E);
+  return ret;
+}
+
+}  // namespace isw
+}  // namespace wcns
