@@ -35,7 +35,21 @@ __global__ void limiter_cert_check_kernel(int kind, const double *__restrict__ r
         Wn[f] = r[f];
         Wt[f] = W0[f] = r[NF + f];
       }
-      cert[i] = tol.hs_implied && state_passes<NDIM>(eos, tol, Wn) && state_passes<NDIM>(eos, tol, Wt);
+      // the sweeps' two routes: from the primitives, then from the state
+      double V[NF];
+      const double ir = 1.0 / (Wt[0] + Wt[1]);
+      double mm = 0.0;
+#pragma unroll
+      for (int k = 0; k < NDIM; ++k) {
+        V[2 + k] = Wt[2 + k] * ir;
+        mm = fma(Wt[2 + k], V[2 + k], mm);
+      }
+      V[0] = Wt[0];
+      V[1] = Wt[1];
+      V[2 + NDIM] = (fma(-0.5, mm, Wt[2 + NDIM]) - mulr(Wt[A], eos.q1)) / mixGamma(eos, Wt[A]);
+      V[A] = Wt[A];
+      cert[i] = tol.hs_implied && state_passes<NDIM>(eos, tol, Wn) &&
+                (primitives_pass<NDIM>(eos, tol, V) || state_passes<NDIM>(eos, tol, Wt));
       const int fl = interp_limit<NDIM>(eos, tol, Wn, Wt);
       exact[i] = fl == 0 && same(Wt, W0);
     } else if (kind == 1) {
