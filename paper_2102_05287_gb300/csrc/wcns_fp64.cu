@@ -77,7 +77,7 @@ __global__ void limiter_cert_check_kernel(int kind, const double *__restrict__ r
         gH[f] = trunc32(f < A ? GHm[f] : f == A ? GHm[A] : GHp[A]);
         eH[f] = 1.9073486328125e-06f * fabsf(gH[f]) + CTINY;
       }
-      cert[i] = tol.hs_implied && flux_certified<NDIM>(eos, tol, l2f, Wi, Wi1, Fi, Fi1, gH, eH, Gm, Gm[A], Gp[A]);
+      cert[i] = tol.hs_implied && flux_certified<NDIM>(eos, tol, l2f, Wi, Wi1, Fi, Fi1, 1, gH, eH, Gm, Gm[A], Gp[A]);
       const int fl = flux_limit<NDIM>(eos, tol, Wi, Wi1, Fi, Fi1, GHm, GHp, lam, Gm, Gp);
       exact[i] = fl == 0 && same(Gm, Gm0) && same(Gp, Gp0);
     } else {
@@ -110,8 +110,8 @@ __global__ void limiter_cert_check_kernel(int kind, const double *__restrict__ r
       // certification, and the FP64 flux with the FP64 limiter
       float gH[NF + 1], eH[NF + 1];
       cert[i] = tol.hs_implied &&
-                hllc1_bound32<NDIM, NDIM - 1>(Wi, vi, pi, ci, Wi1, vr, pr, cr, gH, eH) &&
-                flux_certified<NDIM>(eos, tol, l2f, Wi, Wi1, Fi, Fi1, gH, eH, Gm, Gm[A], Gp[A]);
+                hllc1_bound32<NDIM, NDIM - 1>(Wi, vi, pi, ci, Wi1, vr, pr, cr, 1, gH, eH) &&
+                flux_certified<NDIM>(eos, tol, l2f, Wi, Wi1, Fi, Fi1, 1, gH, eH, Gm, Gm[A], Gp[A]);
       double GH[NF], uH, GHm[NF], GHp[NF];
       hllc<NDIM, NDIM - 1, double>(Wi, vi, pi, Wi[0] + Wi[1], ci, Wi1, vr, pr, Wi1[0] + Wi1[1], cr, GH, uH);
 #pragma unroll
