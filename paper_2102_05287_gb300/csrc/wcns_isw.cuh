@@ -86,13 +86,6 @@ WISW int clz32(unsigned u) {
   return u ? __builtin_clz(u) : 32;
 #endif
 }
-WISW float fdiv(float a, float b) {
-#ifdef __CUDA_ARCH__
-  return __fdividef(a, b);
-#else
-  return a / b;
-#endif
-}
 WISW float frcp(float b) {
 #ifdef __CUDA_ARCH__
   float r;
@@ -102,6 +95,7 @@ WISW float frcp(float b) {
   return 1.0f / b;
 #endif
 }
+WISW float fdiv(float a, float b) { return a * frcp(b); }
 WISW float frsqrt(float b) {
 #ifdef __CUDA_ARCH__
   float r;

@@ -99,47 +99,44 @@ using TileMixed = typename std::conditional<
 // hi = lo = 0 with the sign kept; magnitudes above it give hi = +-inf (NaN
 // stays NaN), lo = 0.
 __device__ __forceinline__ void split_hilo(double v, float &hi, float &lo) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const unsigned int sign = (unsigned int)(b >> 63) << 31;
-  const int e = (int)((b >> 52) & 0x7FFull);
-  const int e32 = e - 1023 + 127;
-  const unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-  if (e32 <= 0 || e32 >= 255) {
-    const unsigned int nan = (e == 0x7FF && m) ? 0x400000u : 0u;
-    hi = __uint_as_float(e32 <= 0 ? sign : (sign | 0x7F800000u | nan));
+  const unsigned int h = (unsigned int)__double2hiint(v), l = (unsigned int)__double2loint(v);
+  const unsigned int sign = h & 0x80000000u, mag = h & 0x7FFFFFFFu;
+  if (mag - 0x38100000u >= 0x0FE00000u) {  // FP32 exponent field outside [1, 254]
+    const unsigned int nan = (mag > 0x7FF00000u || (mag == 0x7FF00000u && l)) ? 0x400000u : 0u;
+    hi = __uint_as_float(mag < 0x38100000u ? sign : (sign | 0x7F800000u | nan));
     lo = 0.0f;
     return;
   }
-  hi = __uint_as_float(sign | ((unsigned int)e32 << 23) | (unsigned int)(m >> 29));
-  const unsigned int low = (unsigned int)(m & 0x1FFFFFFFull);
-  const int es = e - 1075 + 127;  // exponent of the last mantissa bit, biased for FP32
-  const float scale = es > 0 ? __uint_as_float((unsigned int)es << 23) : 0.0f;
-  lo = __uint_as_float(__float_as_uint((float)low * scale) | sign);
+  const unsigned int b = __funnelshift_l(l, mag - 0x38000000u, 3);
+  hi = __uint_as_float(sign | b);
+  // the low 29 bits on the scale of the last one, 2^-52 of hi's binade
+  const int es = (int)(b & 0x7F800000u) - (52 << 23);
+  lo = __uint_as_float(__float_as_uint((float)(l & 0x1FFFFFFFu) * __int_as_float(max(es, 0))) | sign);
 }
 
 // FP32 -> FP64 on the integer pipe (the FP64 pipe is the scarce one):
 // exact for normal numbers, zeros, infinities and NaNs; FP32 subnormals
 // (below 1.2e-38) become zeros of the same sign.
 __device__ __forceinline__ double f2d(float x) {
-  const unsigned int b = __float_as_uint(x);
-  const unsigned int e = (b >> 23) & 0xFFu;
-  const unsigned long long sign = (unsigned long long)(b >> 31) << 63;
-  if (e == 0u) return __longlong_as_double((long long)sign);
-  const unsigned long long e64 = e == 0xFFu ? 0x7FFull : (unsigned long long)(e + 896u);
-  const unsigned long long m = (unsigned long long)(b & 0x7FFFFFu) << 29;
-  return __longlong_as_double((long long)(sign | (e64 << 52) | m));
+  const unsigned int b = __float_as_uint(x), mag = b & 0x7FFFFFFFu;
+  unsigned int h = (mag >> 3) + 0x38000000u, l = b << 29;
+  if (mag - 0x00800000u >= 0x7F000000u) {  // zero or subnormal; infinity or NaN
+    h = mag < 0x00800000u ? 0u : (mag >> 3) | 0x7FF00000u;
+    l = mag < 0x00800000u ? 0u : l;
+  }
+  return __hiloint2double((int)(h | (b & 0x80000000u)), (int)l);
 }
 
 // 1/y for the mixed path's FP64 node work: Newton-Raphson refinement
-// r <- r + r (1 - y r) of an FP32 seed.  The seed, the correctly rounded
-// FP32 reciprocal of y's leading 24 bits, is within ~2^-22 of 1/y; one step
+// r <- r + r (1 - y r) of an FP32 seed.  The seed, the rounded FP32
+// reciprocal of y's leading 24 bits, is within ~2^-22 of 1/y; one step
 // squares that to ~2^-44, far below the FP32 precision the rest of the
 // mixed path carries.  y must be finite, nonzero and within FP32's normal
 // range (densities and Gamma of admissible states are).
 __device__ __forceinline__ double recip_nr(double y) {
   float hi, lo;
   split_hilo(y, hi, lo);
-  const double r = f2d(__frcp_rn(hi));
+  const double r = f2d(fdiv32_rn(1.0f, hi));
   return fma(r, fma(-y, r, 1.0), r);
 }
 
@@ -200,11 +197,11 @@ __device__ __forceinline__ bool rct2_certified(const EosConst &e, const float *x
     m2 += mj * mj;
     dm2 += (2.0f * fabsf(mj) + dm) * dm;
   }
-  const float ke = 0.5f * __fdividef(m2, rho);
-  const float dke = 0.5f * __fdividef(dm2, rlo) + __fdividef(ke * drho, rlo) + margin(ke);
+  const float ke = 0.5f * fdiv32(m2, rho);
+  const float dke = 0.5f * fdiv32(dm2, rlo) + fdiv32(ke * drho, rlo) + margin(ke);
   const float al = x[A];
   const float Gam = e.r2f + e.drf * al;
-  const float pb = __fdividef(e.q1f * al, Gam + 1.0f);
+  const float pb = fdiv32(e.q1f * al, Gam + 1.0f);
   const float dpb = e.q1f * (e.r2f + 1.0f) * margin(mag[A]) + margin(pb);
   const float v = x[E] - ke - pb;
   return v - (margin(mag[E]) + dke + dpb + margin(fabsf(x[E]) + ke + pb)) >= eps;
@@ -497,10 +494,10 @@ __device__ __forceinline__ void sweep_body_mixed(const SweepArgs &a, const Geo &
       // FP32 sound speed: rho c^2 = gbar (p + pbar) (Sec. 2)
       const float a1 = vh[A] + vl[A];
       const float Gam32 = eos.r2f + eos.drf * a1;
-      const float pb32 = __fdividef(eos.q1f * a1, Gam32 + 1.0f);
+      const float pb32 = fdiv32(eos.q1f * a1, Gam32 + 1.0f);
       const float rho32 = vh[0] + vh[1];
       const float pp = vh[E] + vl[E] + pb32;
-      c32 = sqrtf(__fdividef((1.0f + __fdividef(1.0f, Gam32)) * pp, rho32));
+      c32 = sqrtf(fdiv32((1.0f + fdiv32(1.0f, Gam32)) * pp, rho32));
       // Node quantities certified above the limiter tolerances (the first
       // test of Algorithms 1-3); bit set = certified.  hi is the value
       // truncated toward zero, so hi >= eps > 0 implies value >= eps.
@@ -623,8 +620,8 @@ __device__ __forceinline__ void sweep_body_mixed(const SweepArgs &a, const Geo &
       const float ar2 = 0.5f * (hi_i[1] + sm.Vh[1 * T::NN + ni1]);
       const float rb = ar1 + ar2;
       const float cb = 0.5f * (ci + ci1);
-      const float irc = __fdividef(1.0f, rb * cb);
-      const float k1 = ar1 * irc / cb, k2 = ar2 * irc / cb;
+      const float irc = fdiv32(1.0f, rb * cb);
+      const float k1 = fdiv32_rn(ar1 * irc, cb), k2 = fdiv32_rn(ar2 * irc, cb);
       // Steps 2-3 field by field: the projected deviations of two
       // characteristic fields at a time (stencil nodes j = 0..5 are
       // i-2..i+3; node i itself, j = 2, has zero deviation and enters
@@ -682,8 +679,8 @@ __device__ __forceinline__ void sweep_body_mixed(const SweepArgs &a, const Geo &
         const float *Us = side ? UR : UL;
         float *d = dV[side];
         const float dac = Us[NF - 1] - Us[0];
-        d[0] = Us[1] + __fdividef(ar1, 2.0f * cb) * dac;
-        d[1] = Us[2] + __fdividef(ar2, 2.0f * cb) * dac;
+        d[0] = Us[1] + fdiv32(ar1, 2.0f * cb) * dac;
+        d[1] = Us[2] + fdiv32(ar2, 2.0f * cb) * dac;
         int row = 3;
 #pragma unroll
         for (int k = 0; k < NDIM; ++k) {
@@ -704,9 +701,9 @@ __device__ __forceinline__ void sweep_body_mixed(const SweepArgs &a, const Geo &
         const float *d = dV[side];
         const float a1 = ref.a1 + (lo_i[A] + d[A]);
         const float Gam = eos.r2f + eos.drf * a1;
-        const float pb = __fdividef(eos.q1f * a1, Gam + 1.0f);
+        const float pb = fdiv32(eos.q1f * a1, Gam + 1.0f);
         const float rho = ref.rho + (lo_i[0] + lo_i[1] + d[0] + d[1]);
-        cs[side] = sqrtf(__fdividef((1.0f + __fdividef(1.0f, Gam)) * (ref.p + (lo_i[E] + d[E]) + pb), rho));
+        cs[side] = sqrtf(fdiv32((1.0f + fdiv32(1.0f, Gam)) * (ref.p + (lo_i[E] + d[E]) + pb), rho));
       }
       // Interpolation limiter (Sec. 5.1): FP32 certification, else FP64.
       if (a.scheme == SCHEME_PP) {
@@ -722,7 +719,7 @@ __device__ __forceinline__ void sweep_body_mixed(const SweepArgs &a, const Geo &
             const float om = ((1.0f - hi_i[A]) - lo_i[A]) - d[A];
             const float pt = hi_i[E] + (lo_i[E] + d[E]);
             const float Gam = eos.r2f + eos.drf * al;
-            const float pb = __fdividef(eos.q1f * al, Gam + 1.0f);
+            const float pb = fdiv32(eos.q1f * al, Gam + 1.0f);
             cert = r1 - margin(fabsf(hi_i[0]) + fabsf(d[0])) >= epsf_ar &&
                    r2 - margin(fabsf(hi_i[1]) + fabsf(d[1])) >= epsf_ar &&
                    al - margin(fabsf(hi_i[A]) + fabsf(d[A])) >= epsf_a &&
