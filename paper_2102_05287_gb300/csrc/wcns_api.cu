@@ -55,17 +55,18 @@ namespace {
 // max over cells of (|u_d| + c) (Sec. 3.3) into ctl->smax[slot][d].
 __global__ void reduce_wavespeed_kernel(const double *__restrict__ W, long long N, int ndim,
                                         EosConst e, StepCtl *ctl, int slot) {
-  double smax[3] = {0.0, 0.0, 0.0};
+  // bit patterns: |u_d| + c >= 0 or a NaN, which orders above every number
+  unsigned long long smax[3] = {0ull, 0ull, 0ull};
   const int E = 2 + ndim, A = 3 + ndim;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N;
        i += (long long)gridDim.x * blockDim.x) {
     double m[3], sp[3];
     for (int j = 0; j < ndim; ++j) m[j] = W[(2 + j) * N + i];
     state_wavespeeds(W[i], W[N + i], m, W[E * N + i], W[A * N + i], ndim, e, sp);
-    for (int j = 0; j < ndim; ++j) smax[j] = (sp[j] > smax[j] || sp[j] != sp[j]) ? sp[j] : smax[j];
+    for (int j = 0; j < ndim; ++j) smax[j] = max(smax[j], (unsigned long long)__double_as_longlong(sp[j]));
   }
   for (int j = 0; j < ndim; ++j) {
-    unsigned long long b = __double_as_longlong(smax[j]);
+    unsigned long long b = smax[j];
     for (int o = 16; o > 0; o >>= 1) {
       const unsigned long long ob = __shfl_xor_sync(0xffffffffu, b, o);
       b = ob > b ? ob : b;

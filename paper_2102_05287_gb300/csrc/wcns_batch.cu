@@ -106,15 +106,15 @@ __global__ void batch_reduce_kernel(const double *__restrict__ W, long long tota
     const int prob = b.tile_prob[t];
     const int first = b.tile_first[t];
     const int n = b.ncell[prob];
-    double smax = 0.0;
+    unsigned long long smax = 0ull;  // bit patterns: a NaN orders above every number
     for (int i = first + threadIdx.x; i < min(first + tile_cells, n); i += blockDim.x) {
       const long long idx = b.offsets[prob] + i;
       const double m = W[2 * total + idx];
       double s;
       state_wavespeeds(W[idx], W[total + idx], &m, W[3 * total + idx], W[4 * total + idx], 1, e, &s);
-      smax = (s > smax || s != s) ? s : smax;
+      smax = max(smax, (unsigned long long)__double_as_longlong(s));
     }
-    unsigned long long bits = __double_as_longlong(smax);
+    unsigned long long bits = smax;
     for (int o = 16; o > 0; o >>= 1) {
       const unsigned long long ob = __shfl_xor_sync(0xffffffffu, bits, o);
       bits = ob > bits ? ob : bits;
@@ -270,7 +270,7 @@ __global__ void batch2_reduce_kernel(const double *__restrict__ W, long long tot
   for (int t = blockIdx.x; t < b.ntiles; t += gridDim.x) {
     const int prob = b.tile_prob[t];
     const int nx = b.nx[prob], ny = b.ny[prob];
-    double smax[2] = {0.0, 0.0};
+    unsigned long long smax[2] = {0ull, 0ull};
     for (int q = threadIdx.x; q < T::TL * (T::TM - 1); q += blockDim.x) {
       const int y = b.tile_line[t] + q / (T::TM - 1);
       const int x = b.tile_first[t] + q % (T::TM - 1);
@@ -279,10 +279,10 @@ __global__ void batch2_reduce_kernel(const double *__restrict__ W, long long tot
       const double m[2] = {W[2 * total + idx], W[3 * total + idx]};
       double sp[2];
       state_wavespeeds(W[idx], W[total + idx], m, W[4 * total + idx], W[5 * total + idx], 2, e, sp);
-      for (int j = 0; j < 2; ++j) smax[j] = (sp[j] > smax[j] || sp[j] != sp[j]) ? sp[j] : smax[j];
+      for (int j = 0; j < 2; ++j) smax[j] = max(smax[j], (unsigned long long)__double_as_longlong(sp[j]));
     }
     for (int j = 0; j < 2; ++j) {
-      unsigned long long bits = __double_as_longlong(smax[j]);
+      unsigned long long bits = smax[j];
       for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long ob = __shfl_xor_sync(0xffffffffu, bits, o);
         bits = ob > bits ? ob : bits;
