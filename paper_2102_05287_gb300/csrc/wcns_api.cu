@@ -52,27 +52,87 @@ namespace {
 // ---------------------------------------------------------------------------
 // Device helpers.
 // ---------------------------------------------------------------------------
-// max over cells of (|u_d| + c) (Sec. 3.3) into ctl->smax[slot][d].
-__global__ void reduce_wavespeed_kernel(const double *__restrict__ W, long long N, int ndim,
-                                        EosConst e, StepCtl *ctl, int slot) {
+// FP32 upper bound of |u_d| + c of one conservative state for every d: true
+// with c and 1/rho set where it holds.  The operands are truncated images
+// (within 2^-20); the margins cover that and the FP32 roundings: 2^-18 of the
+// terms of rho ctilde^2 = E - |m|^2 / (2 rho) - pbar, Gamma from below, and
+// 1e-5 in the end.  False where the state is not clearly admissible.
+__device__ __forceinline__ bool wavespeed_bound(double a1r1, double a2r2, const double *m, double E, double a1,
+                                                int ndim, const EosConst &e, float &c, float &ir) {
+  const float rho = trunc32(a1r1) + trunc32(a2r2), al = trunc32(a1), En = trunc32(E);
+  float m2 = 0.0f;
+  for (int j = 0; j < ndim; ++j) {
+    const float v = trunc32(m[j]);
+    m2 = fmaf(v, v, m2);
+  }
+  const float G = fmaf(e.drf, al, e.r2f), Gl = G - 4e-6f * (fabsf(e.drf) * al + fabsf(e.r2f));
+  if (!(rho > 1e-30f && al >= 0.0f && al <= 1.0f && Gl > 0.0f)) return false;
+  ir = __fdividef(1.00001f, rho);
+  const float ke = 0.5f * m2 * ir, pb = __fdividef(e.q1f * al, G + 1.0f), iG = __fdividef(1.0f, Gl);
+  const float rct = En - ke - pb, err = 2e-5f * (fabsf(En) + ke + pb);
+  c = sqrtf((1.0f + iG) * iG * (rct + err) * ir);
+  return rct > err && c < 1e30f;
+}
+
+// max over cells of (|u_d| + c) (Sec. 3.3) into ctl->smax[slot][d].  A thread's
+// first cell goes through the FP64 evaluation and its warp publishes the
+// maximum; a later cell does only where its FP32 upper bound reaches the
+// maxima read after that or found by the thread since, so that the FP64 pipe, which bounded the reduction (256^3:
+// 0.81 ms), works on few cells of a state that is not uniform (0.25 ms).
+template <int ndim>
+__global__ void reduce_wavespeed_kernel(const double *__restrict__ W, long long N, EosConst e, StepCtl *ctl, int slot) {
   // bit patterns: |u_d| + c >= 0 or a NaN, which orders above every number
   unsigned long long smax[3] = {0ull, 0ull, 0ull};
-  const int E = 2 + ndim, A = 3 + ndim;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-       i += (long long)gridDim.x * blockDim.x) {
-    double m[3], sp[3];
-    for (int j = 0; j < ndim; ++j) m[j] = W[(2 + j) * N + i];
-    state_wavespeeds(W[i], W[N + i], m, W[E * N + i], W[A * N + i], ndim, e, sp);
-    for (int j = 0; j < ndim; ++j) smax[j] = max(smax[j], (unsigned long long)__double_as_longlong(sp[j]));
-  }
-  for (int j = 0; j < ndim; ++j) {
-    unsigned long long b = smax[j];
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long ob = __shfl_xor_sync(0xffffffffu, b, o);
-      b = ob > b ? ob : b;
+  float top[3] = {0.0f, 0.0f, 0.0f};  // known maxima, rounded down
+  constexpr int E = 2 + ndim, A = 3 + ndim;
+  auto publish = [&]() {
+    for (int j = 0; j < ndim; ++j) {
+      unsigned long long b = smax[j];
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, b, o);
+        b = ob > b ? ob : b;
+      }
+      if ((threadIdx.x & 31) == 0 && b) atomicMax(&ctl->smax[slot][j], b);
     }
-    if ((threadIdx.x & 31) == 0 && b) atomicMax(&ctl->smax[slot][j], b);
+  };
+  const long long stride = (long long)gridDim.x * blockDim.x, first = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  for (long long base = 0; base < N; base += stride) {
+    const long long i = base + first;
+    if (i < N) {
+      double m[3], sp[3];
+      for (int j = 0; j < ndim; ++j) m[j] = W[(2 + j) * N + i];
+      const double r1 = W[i], r2 = W[N + i], En = W[E * N + i], a1 = W[A * N + i];
+      float c, ir;
+      bool below = base > 0 && wavespeed_bound(r1, r2, m, En, a1, ndim, e, c, ir);
+      if (below)
+        for (int j = 0; j < ndim; ++j) {
+          // a NaN maximum lets nothing stay below it and stays the maximum
+          below = below && 1.00001f * fmaf(fabsf(trunc32(m[j])), ir, c) < top[j];
+        }
+      if (!below) {
+        state_wavespeeds(r1, r2, m, En, a1, ndim, e, sp);
+        for (int j = 0; j < ndim; ++j) {
+          smax[j] = max(smax[j], (unsigned long long)__double_as_longlong(sp[j]));
+          top[j] = fmaxf(top[j], trunc32(sp[j]));
+        }
+      }
+    }
+    if (base == 0 && stride < N) {
+      publish();
+      for (int j = 0; j < ndim; ++j) top[j] = trunc32(__longlong_as_double((long long)__ldcg(&ctl->smax[slot][j])));
+    }
   }
+  publish();
+}
+
+cudaError_t launch_reduce_wavespeed(int blocks, const double *W, long long N, int ndim, const EosConst &e, StepCtl *ctl,
+                                    int slot, cudaStream_t st) {
+  switch (ndim) {
+    case 1: reduce_wavespeed_kernel<1><<<blocks, 256, 0, st>>>(W, N, e, ctl, slot); break;
+    case 2: reduce_wavespeed_kernel<2><<<blocks, 256, 0, st>>>(W, N, e, ctl, slot); break;
+    default: reduce_wavespeed_kernel<3><<<blocks, 256, 0, st>>>(W, N, e, ctl, slot); break;
+  }
+  return cudaGetLastError();
 }
 
 // The uniform Dirichlet ghost states of a handle, passed BY VALUE as a
@@ -159,9 +219,9 @@ int launch_reduce(wcns_handle *h, const double *W, int slot) {
   long long blocks = (h->N + threads - 1) / threads;
   if (blocks > 152 * 8) blocks = 152 * 8;
   if (blocks < 1) blocks = 1;
-  reduce_wavespeed_kernel<<<(int)blocks, threads, 0, h->launch_stream>>>(W, h->N, h->ndim, h->eos, h->ctl, slot);
   h->launches++;
-  return cuda_status(cudaGetLastError());
+  return cuda_status(
+      launch_reduce_wavespeed((int)blocks, W, h->N, h->ndim, h->eos, h->ctl, slot, h->launch_stream));
 }
 
 int launch_init(wcns_handle *h, double t, double t_end) {
@@ -351,8 +411,7 @@ int update_bc_wavespeed(wcns_handle *h) {
       }
       const long long n = h->N / h->n[d];
       const long long blocks = (n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024;
-      reduce_wavespeed_kernel<<<(int)blocks, 256, 0, st>>>(src, n, h->ndim, h->eos, h->ctl, 0);
-      e = cudaGetLastError();
+      e = launch_reduce_wavespeed((int)blocks, src, n, h->ndim, h->eos, h->ctl, 0, st);
     }
   }
   if (e == cudaSuccess && u.count) {
