@@ -287,7 +287,9 @@ def fp64_roofline(ops, peaks, avg_ms, ncell, kernel):
                     "min/max, division and square root one flop each, x cells of one launch, over the launch's "
                     "live CUDA-event time; peak = the FP64 FMA rate of this GPU measured live (of measured). "
                     "frac_div_sqrt_weighted counts each division / square root at its measured cost in "
-                    "FMA-flops (%.1f / %.1f)" % (div_eq, sqrt_eq)}
+                    "FMA-flops (%.1f / %.1f).  A fraction above 1 means that part of these flops does not run "
+                    "on the FP64 pipe: the sweeps evaluate the IS weights, the HCS combination and the idle "
+                    "limiters' tests on the FP32 and integer pipes to FP64 accuracy" % (div_eq, sqrt_eq)}
 
 
 # ---------------------------------------------------------------------------

@@ -83,7 +83,11 @@ typedef struct {
 
 /* Precision of the hot path. */
 enum {
-  WCNS_FP64 = 0,   /* every step in FP64 */
+  WCNS_FP64 = 0,   /* every step to FP64 accuracy: states, fluxes, limiters and their
+                      sums in FP64; the WCNS-IS weights' correction in FP32 or pairs of
+                      FP32 values where a bound certifies it to a quarter of the
+                      result's FP64 rounding (FP64 elsewhere), linear combinations of
+                      node values in exact integers */
   WCNS_MIXED = 1   /* FP32 characteristic projection, WCNS-IS interpolation and
                       HLLC fluxes; FP64 pressure / sound speed, limiter
                       blending-coefficient solve and state accumulation */
