@@ -174,6 +174,7 @@ __global__ void init_ctl_kernel(StepCtl *ctl, const DevStats *stats, double t, d
 // tau_d, Sec. 3.3), clip to t_end, and clear the accumulators of the stages.
 __global__ void step_begin_kernel(StepCtl *ctl, int ndim, double ix0, double ix1, double ix2,
                                   double dt_fixed, double cfl, int advance_time) {
+  after_predecessor();
   const double ix[3] = {ix0, ix1, ix2};
   double tsum = 0.0;
   for (int d = 0; d < 3; ++d) {
@@ -231,10 +232,9 @@ int launch_init(wcns_handle *h, double t, double t_end) {
 }
 
 int launch_begin(wcns_handle *h, double dt_fixed, double cfl, int advance_time) {
-  step_begin_kernel<<<1, 1, 0, h->launch_stream>>>(h->ctl, h->ndim, h->inv_dx[0], h->inv_dx[1], h->inv_dx[2],
-                                            dt_fixed, cfl, advance_time);
   h->launches++;
-  return cuda_status(cudaGetLastError());
+  return cuda_status(launch_after(step_begin_kernel, dim3(1, 1, 1), 1, 0, h->launch_stream, true, h->ctl, h->ndim,
+                                  h->inv_dx[0], h->inv_dx[1], h->inv_dx[2], dt_fixed, cfl, advance_time));
 }
 
 // The k-th sweep direction of an RHS evaluation: x, y, z in FP64; in the

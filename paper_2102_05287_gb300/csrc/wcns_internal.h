@@ -118,6 +118,36 @@ inline int status_from_counts(const StepCtl &c, const DevStats &s, int ok, int e
 }
 
 #ifdef __CUDACC__
+// Launch latency between the kernels of a step: a kernel launched with
+// `early` may be scheduled while its predecessor on the stream still runs
+// (programmatic stream serialization).  after_predecessor() is the first
+// statement of such a kernel: it waits for the predecessor's end and its
+// writes (at once in an ordinary launch), then lets the successor be
+// scheduled.  Only for grids whose blocks are all resident with room to
+// spare: waiting blocks of a large grid would hold the predecessor's slots.
+// One step of a 200-cell FP64 shock tube 124 -> 119.5 us, ten of a 512-cell run
+// 551 -> 530 us.
+constexpr long long EARLY_MAX_BLOCKS = 304;
+__device__ __forceinline__ void after_predecessor() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool early,
+                         A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // |u_d| + c of one conservative state for d < ndim (Sec. 3.3), with the FP64
 // mixture thermodynamics of Sec. 2: c^2 = ((Gamma + 1) rho e - Pi) / (Gamma^2
 // rho).  Every FP64 reduction of max(|u_d| + c) (single grids, Dirichlet

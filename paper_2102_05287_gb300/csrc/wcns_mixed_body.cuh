@@ -1020,6 +1020,7 @@ __global__ void __launch_bounds__(T::THREADS,
                                                          : MIXED_MIN_BLOCKS))
     sweep_kernel_mixed(const SweepArgs a) {
   extern __shared__ double smem_raw[];
+  after_predecessor();
   if (!a.ctl->active) return;
   sweep_body_mixed<NDIM, DIR, T>(a, GridGeo<NDIM, DIR, T>(a), smem_raw);
 }
@@ -1037,8 +1038,9 @@ cudaError_t launch_sweep_mixed_t(const SweepArgs &a, cudaStream_t st) {
     return r;
   });
   if (e != cudaSuccess) return e;
-  sweep_kernel_mixed<NDIM, DIR, T><<<sweep_grid<DIR, T>(a), T::THREADS, bytes, st>>>(a);
-  return cudaGetLastError();
+  const dim3 g = sweep_grid<DIR, T>(a);
+  return launch_after(sweep_kernel_mixed<NDIM, DIR, T>, g, T::THREADS, bytes, st,
+                      (long long)g.x * g.y * g.z <= EARLY_MAX_BLOCKS, a);
 }
 
 
