@@ -434,8 +434,10 @@ __device__ __forceinline__ void sweep_body_mixed(const SweepArgs &a, const Geo &
       }
     } else {
       idx = ln.base + (long long)src * ln.stride;
+      // ordinary loads, as in sweep_body: a predecessor may still write W_in
+      // when this kernel is launched
 #pragma unroll
-      for (int f = 0; f < NF; ++f) w[f] = __ldg(a.W_in + (long long)f * N + idx);
+      for (int f = 0; f < NF; ++f) w[f] = a.W_in[(long long)f * N + idx];
       if (flip) w[2 + DIR] = -w[2 + DIR];
     }
     // Sec. 2 in FP64: p from rho e (the p + p_inf cancellation).  The later
