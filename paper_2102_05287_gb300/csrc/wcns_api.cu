@@ -55,8 +55,9 @@ namespace {
 // FP32 upper bound of |u_d| + c of one conservative state for every d: true
 // with c and 1/rho set where it holds.  The operands are truncated images
 // (within 2^-20); the margins cover that and the FP32 roundings: 2^-18 of the
-// terms of rho ctilde^2 = E - |m|^2 / (2 rho) - pbar, Gamma from below, and
-// 1e-5 in the end.  False where the state is not clearly admissible.
+// terms of rho ctilde^2 = E - |m|^2 / (2 rho) - pbar, Gamma from below in 1/Gamma
+// and from above in pbar = Pi / (Gamma + 1) (its two terms can be much larger
+// than their sum), and 1e-5 in the end.  False where the state is not clearly admissible.
 __device__ __forceinline__ bool wavespeed_bound(double a1r1, double a2r2, const double *m, double E, double a1,
                                                 int ndim, const EosConst &e, float &c, float &ir) {
   const float rho = trunc32(a1r1) + trunc32(a2r2), al = trunc32(a1), En = trunc32(E);
@@ -65,11 +66,11 @@ __device__ __forceinline__ bool wavespeed_bound(double a1r1, double a2r2, const 
     const float v = trunc32(m[j]);
     m2 = fmaf(v, v, m2);
   }
-  const float G = fmaf(e.drf, al, e.r2f), Gl = G - 4e-6f * (fabsf(e.drf) * al + fabsf(e.r2f));
+  const float G = fmaf(e.drf, al, e.r2f), dG = 4e-6f * (fabsf(e.drf) * al + fabsf(e.r2f)), Gl = G - dG;
   if (!(rho > 1e-30f && al >= 0.0f && al <= 1.0f && Gl > 0.0f)) return false;
   ir = __fdividef(1.00001f, rho);
   const float ke = 0.5f * m2 * ir, pb = __fdividef(e.q1f * al, G + 1.0f), iG = __fdividef(1.0f, Gl);
-  const float rct = En - ke - pb, err = 2e-5f * (fabsf(En) + ke + pb);
+  const float rct = En - ke - pb, err = 2e-5f * (fabsf(En) + ke + pb) + pb * __fdividef(dG, G + 1.0f);
   c = sqrtf((1.0f + iG) * iG * (rct + err) * ir);
   return rct > err && c < 1e30f;
 }
