@@ -57,17 +57,20 @@ namespace {
 // (within 2^-20); the margins cover that and the FP32 roundings: 2^-18 of the
 // terms of rho ctilde^2 = E - |m|^2 / (2 rho) - pbar, Gamma from below in 1/Gamma
 // and from above in pbar = Pi / (Gamma + 1) (its two terms can be much larger
-// than their sum), and 1e-5 in the end.  False where the state is not clearly admissible.
+// than their sum), and 1e-5 in the end.  False where the state is not clearly
+// admissible (partial densities of opposite signs lose digits in their sum),
+// and for densities whose reciprocal leaves FP32's range (__fdividef gives 0
+// above 2^126) or makes a momentum count that truncates to zero.
 __device__ __forceinline__ bool wavespeed_bound(double a1r1, double a2r2, const double *m, double E, double a1,
                                                 int ndim, const EosConst &e, float &c, float &ir) {
-  const float rho = trunc32(a1r1) + trunc32(a2r2), al = trunc32(a1), En = trunc32(E);
+  const float d1 = trunc32(a1r1), d2 = trunc32(a2r2), rho = d1 + d2, al = trunc32(a1), En = trunc32(E);
   float m2 = 0.0f;
   for (int j = 0; j < ndim; ++j) {
     const float v = trunc32(m[j]);
     m2 = fmaf(v, v, m2);
   }
   const float G = fmaf(e.drf, al, e.r2f), dG = 4e-6f * (fabsf(e.drf) * al + fabsf(e.r2f)), Gl = G - dG;
-  if (!(rho > 1e-30f && al >= 0.0f && al <= 1.0f && Gl > 0.0f)) return false;
+  if (!(d1 >= 0.0f && d2 >= 0.0f && rho > 1e-10f && rho < 1e30f && al >= 0.0f && al <= 1.0f && Gl > 0.0f)) return false;
   ir = __fdividef(1.00001f, rho);
   const float ke = 0.5f * m2 * ir, pb = __fdividef(e.q1f * al, G + 1.0f), iG = __fdividef(1.0f, Gl);
   const float rct = En - ke - pb, err = 2e-5f * (fabsf(En) + ke + pb) + pb * __fdividef(dG, G + 1.0f);
@@ -78,8 +81,9 @@ __device__ __forceinline__ bool wavespeed_bound(double a1r1, double a2r2, const 
 // max over cells of (|u_d| + c) (Sec. 3.3) into ctl->smax[slot][d].  A thread's
 // first cell goes through the FP64 evaluation and its warp publishes the
 // maximum; a later cell does only where its FP32 upper bound reaches the
-// maxima read after that or found by the thread since, so that the FP64 pipe, which bounded the reduction (256^3:
-// 0.81 ms), works on few cells of a state that is not uniform (0.25 ms).
+// maxima read after that or found by the thread since, so that the FP64 pipe,
+// which bounded the reduction (256^3: 0.81 ms), works on few cells of a state
+// that is not uniform (0.25 ms).
 template <int ndim>
 __global__ void reduce_wavespeed_kernel(const double *__restrict__ W, long long N, EosConst e, StepCtl *ctl, int slot) {
   // bit patterns: |u_d| + c >= 0 or a NaN, which orders above every number

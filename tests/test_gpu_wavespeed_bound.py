@@ -1,10 +1,12 @@
 """max(|u_d| + c): the reduction's FP32 screening must not pass over the cell
 that holds the maximum, for every gas that wcns_create accepts.  One faster cell
-at the end of a grid of equal ones, whose maximum every thread knows by then, in
-a gas with gamma_g near 1, whose Gamma = dr alpha1 + r2 is a small difference
-of large numbers near alpha1 = 1, near rho c^2 = 0, where pbar's error in FP32
-can exceed E - pbar (without an allowance the speed comes out up to 25 % low
-for gamma_g = 1.0003).
+at the end of a grid of equal ones, whose maximum every thread knows by then:
+- a gas with gamma_g near 1, whose Gamma = dr alpha1 + r2 is a small difference
+  of large numbers near alpha1 = 1, near rho c^2 = 0, where pbar's error in
+  FP32 can exceed E - pbar (without an allowance the speed comes out up to 25 %
+  low for gamma_g = 1.0003);
+- densities and energies at the ends of FP32's range, and partial densities
+  whose sum cancels.
 The faster cell is 1 % ahead.  A grid of that one cell is not screened, so the
 two results have to be equal."""
 import numpy as np
@@ -51,3 +53,12 @@ def test_gamma_near_one(gamma_g):
         for c in (20.0, 34.0, 60.0):
             got, want = fastest(gamma_g, float(a1), 1000.0, 1e-5, 0.0, c)
             assert got == want, (a1, c, got, want)
+
+
+@pytest.mark.parametrize("rho1, rho2, m, c", [(0.0, 1e38, 0.0, 1.0), (0.0, 2e38, 1e38, 0.5), (0.0, 1e31, 1e30, 3e3),
+                                             (0.0, 1e-25, 1e-30, 1e3), (0.0, 1e-30, 1e-38, 1e-9),
+                                             (0.0, 1e-12, 1e-20, 1e7), (1.0, -0.9999999, 0.0, 10.0)])
+def test_densities_at_the_ends_of_fp32(rho1, rho2, m, c):
+    # alpha1 = 0: pbar = 0, so that c is free
+    got, want = fastest(1.4, 0.0, rho1, rho2, m, c)
+    assert got == want, (got, want)
