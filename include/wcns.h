@@ -84,10 +84,13 @@ typedef struct {
 /* Precision of the hot path. */
 enum {
   WCNS_FP64 = 0,   /* every step to FP64 accuracy: states, fluxes, limiters and their
-                      sums in FP64; the WCNS-IS weights' correction in FP32 or pairs of
-                      FP32 values where a bound certifies it to a quarter of the
-                      result's FP64 rounding (FP64 elsewhere), linear combinations of
-                      node values in exact integers */
+                      sums in FP64; linear combinations of node values in integers,
+                      cut at 2^-54 of the largest; the WCNS-IS weights' correction in
+                      FP32 or pairs of FP32 values where its error is at most 2^-54
+                      (s + |u|), u the interpolated deviation, and in FP64 elsewhere.
+                      s is the node's value for densities and alpha1; for velocities
+                      |v| + the stencil's largest deviation (its binade), and for the
+                      acoustic fields |p| / (rho c) more, if the pressure varies */
   WCNS_MIXED = 1   /* FP32 characteristic projection, WCNS-IS interpolation and
                       HLLC fluxes; FP64 pressure / sound speed, limiter
                       blending-coefficient solve and state accumulation */

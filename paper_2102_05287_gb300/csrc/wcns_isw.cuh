@@ -324,11 +324,12 @@ WISW int64_t corr_int(F2 c) {
 
 // WCNS-IS of the deviations um2, um1, (0), up1, up2, up3 of nodes i-2 .. i+3
 // from node i: left-biased value ul and right-biased value ur at i+1/2.
-// e4: 4 eps.  scale: the magnitude whose rounding the result may carry.
+// e4: 4 eps.  scale: the magnitude whose rounding the result may carry: scl,
+// and own times the largest deviation's binade / UNIT.
 // Bit 0 / 1 set: ul / ur is within 2^-54 (scale + |u|) of the exact value
 // plus the fixed-point rounding; clear: not decided.  bit 2: pairs used.
 WISW int interpolate(double um2, double um1, double up1, double up2, double up3, double e4, float scl, double &ul,
-                     double &ur) {
+                     double &ur, float own = 0.0f) {
   unsigned mx = hi32(um2) & 0x7FFFFFFFu, t;
   t = hi32(um1) & 0x7FFFFFFFu;
   mx = t > mx ? t : mx;
@@ -353,7 +354,7 @@ WISW int interpolate(double um2, double um1, double up1, double up2, double up3,
   const float eps = ee < -100 ? 0.0f : from_bits32(((unsigned)(ee + 127) << 23) | ((eh & 0xFFFFFu) << 3) | (lo32(e4) >> 29));
   int es = 1022 - E + 22;
   es = es > 100 ? 100 : (es < -120 ? -120 : es);
-  const float sc = scl * from_bits32((unsigned)(es + 127) << 23);
+  const float sc = fmaf(scl, from_bits32((unsigned)(es + 127) << 23), own);
   const float mtol = 2.3283064365386963e-10f;  // 2^-54 UNIT
   int ret = 0;
   // one loop body for the two sides: unrolled, the code's fetch cost 8 % of a

@@ -74,3 +74,11 @@ def test_no_less_accurate_than_the_fp64_formula(tmp_path, fam):
     new, fp64, decided = figures(build(tmp_path, "(float)(fabs(z) + md)", ""), fam)
     assert decided > 0.3
     assert new <= 1.01 * fp64, (new, fp64)
+
+
+@pytest.mark.parametrize("fam", range(len(FAMILIES)), ids=FAMILIES)
+def test_velocities_no_less_accurate_than_the_fp64_formula(tmp_path, fam):
+    """As the sweeps call it for a velocity: the value, and own = UNIT."""
+    new, fp64, decided = figures(build(tmp_path, "(float)fabs(z)", ", wcns::isw::UNIT"), fam)
+    assert decided > 0.3
+    assert new <= 1.01 * fp64, (new, fp64)
