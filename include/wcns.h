@@ -373,8 +373,8 @@ int wcns_batch_set_options(wcns_batch *b, const wcns_options *opt);
  * W_packed).  Each stage is one persistent launch over all problems; one
  * step (dt update + three stages) is captured once into a CUDA graph and
  * replayed.  The first call tunes the tile length (63, 127 or 255 cells)
- * and the persistent grid (1, 2, 4 or 8 blocks per SM; 2D: 1 up to the
- * occupancy limit) by timing trial steps on the tuning copy; make it
+ * and the persistent grid (blocks per SM from the occupancy limit down in
+ * halves) by timing trial steps on the tuning copy; make it
  * before any stream capture of the
  * caller's.  t_out: optional DEVICE array of nprob doubles; each problem's
  * step sizes are added to it.  Ordered after the caller's pending work on
