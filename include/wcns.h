@@ -296,6 +296,21 @@ int wcns_check_division(const double *a, const double *b, double *q, long long n
  * kind, n < 0 or missing arrays. */
 int wcns_check_math(int kind, const double *a, const double *b, double *q, long long n, void *stream);
 
+/* Verification aid (not part of the method): the FP64 sweeps' evaluation of
+ * WCNS-IS (Sec. 4.3) in integers and FP32 on n stencils.  Row i of the DEVICE
+ * array rows (8 n doubles): the deviations of nodes i-2, i-1, i+1, i+2, i+3
+ * from node i; 4 eps; s, the magnitude whose FP64 rounding the result may
+ * carry; and w, 1 if that includes the largest deviation's binade (the
+ * sweeps' velocities), else 0, as multiples of 2^22 (0 or 4194304).  u (2 n
+ * doubles): left- and right-biased deviation at i+1/2; decided (n ints): bit
+ * 0 / 1 set where the left / right one is accepted: then its distance to the
+ * exact value is at most 2^-54 (s + w 2^-22 B + |u|), plus 2.8 * 2^-54 B for
+ * the integers' cut at 2^-54 of B, the power of two above the largest
+ * deviation, plus the rounding of u; clear where the sweeps evaluate the
+ * formula in FP64 instead; bit 2: in pairs of FP32 values.  Asynchronous on
+ * `stream`.  WCNS_E_INVALID_ARG for n < 0 or missing arrays. */
+int wcns_check_interp(const double *rows, double *u, int *decided, long long n, void *stream);
+
 /* Verification aid (not part of the method): the FP64 sweeps skip the
  * limiters of Secs. 5.1-5.2 (Algorithms 1-6) where an FP32 test from
  * truncated operands, with a rigorous error margin, certifies that every

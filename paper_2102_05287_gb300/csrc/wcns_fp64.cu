@@ -20,6 +20,14 @@ __global__ void math_check_kernel(int kind, const double *__restrict__ a, const 
     q[i] = kind == 0 ? rcp_nr(a[i]) : kind == 1 ? sqrt_nr(a[i]) : sqrt_ratio(a[i], b[i]);
 }
 
+__global__ void interp_check_kernel(const double *__restrict__ rows, double *__restrict__ u, int *__restrict__ decided,
+                                    long long n) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const double *r = rows + 8 * i;
+    decided[i] = isw::interpolate(r[0], r[1], r[2], r[3], r[4], r[5], (float)r[6], u[2 * i], u[2 * i + 1], (float)r[7]);
+  }
+}
+
 // One case per thread: the sweeps' certification decision and the FP64
 // limiter's outcome on the same inputs (row layouts as in wcns.h).
 template <int NDIM>
@@ -173,5 +181,13 @@ extern "C" int wcns_check_math(int kind, const double *a, const double *b, doubl
   if (n == 0) return WCNS_OK;
   const long long blocks = (n + 255) / 256 < 152 * 8 ? (n + 255) / 256 : 152 * 8;
   wcns::math_check_kernel<<<(int)blocks, 256, 0, (cudaStream_t)stream>>>(kind, a, b, q, n);
+  return cudaGetLastError() == cudaSuccess ? WCNS_OK : WCNS_E_CUDA;
+}
+
+extern "C" int wcns_check_interp(const double *rows, double *u, int *decided, long long n, void *stream) {
+  if (n < 0 || (n > 0 && (!rows || !u || !decided))) return WCNS_E_INVALID_ARG;
+  if (n == 0) return WCNS_OK;
+  const long long blocks = (n + 127) / 128 < 152 * 8 ? (n + 127) / 128 : 152 * 8;
+  wcns::interp_check_kernel<<<(int)blocks, 128, 0, (cudaStream_t)stream>>>(rows, u, decided, n);
   return cudaGetLastError() == cudaSuccess ? WCNS_OK : WCNS_E_CUDA;
 }
