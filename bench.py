@@ -228,18 +228,25 @@ MIXED_FP64_STEPS = ("node_eos", "node_flux", "update", "ssprk3_combine")
 PROFILE_STEPS_MIXED = 5
 
 
-def mixed_roofline(ops, peaks, avg_ms, ncell, fallbacks):
-    """Roofline of the dominant mixed sweep: algorithmic FP64 flops at the
-    FP64 FMA peak plus FP32 flops at the FP32 FMA peak (divisions and square
-    roots as one flop each); the 'overlapped' form takes the larger of the
-    two times instead of their sum."""
+# The FP64 sweeps' steps on the FP64 pipe.  The others run on the FP32 and
+# integer pipes to FP64 accuracy: the IS weights, the HCS combination, and the
+# idle limiters' tests with their first-order flux.
+FP64_PIPE_STEPS = ("node_eos", "node_flux", "projection", "back_projection", "midpoint_hllc", "update",
+                   "ssprk3_combine", "max_wavespeed")
+
+
+def two_pipes(ops, peaks, avg_ms, ncell, fp64_steps):
+    """Algorithmic flops of the steps fp64_steps at the FP64 FMA peak plus
+    those of the others at the FP32 FMA peak (divisions and square roots as
+    one flop each); the 'overlapped' form takes the larger of the two times
+    instead of their sum."""
     f64 = f32 = 0.0
     for step, c in ops["per_step"].items():
         n = c["add"] + c["mul"] + c["div"] + c["sqrt"] + c["minmax"]
-        if step in MIXED_FP64_STEPS:
+        if step in fp64_steps:
             f64 += n
         else:
-            f32 += n  # the wave-speed maximum included: reduced in FP32 in the combine epilogue
+            f32 += n
     p64 = peaks.get("fp64_fma_tflops", 1.25) * 1e12
     p32 = peaks.get("fp32_fma_tflops", 76.5) * 1e12
     t64 = f64 * ncell / p64
@@ -252,44 +259,52 @@ def mixed_roofline(ops, peaks, avg_ms, ncell, fallbacks):
             "frac": (t64 + t32) / t, "frac_overlapped": max(t64, t32) / t,
             "fp64_flops_per_cell_dir": f64, "fp32_flops_per_cell_dir": f32,
             "roofline_us": (t64 + t32) * 1e6, "roofline_us_overlapped": max(t64, t32) * 1e6,
-            "avg_launch_ms": avg_ms, "fp64_fallbacks": fallbacks, "traffic": None,
-            "note": "mixed sweep: FP64 steps %s at the measured FP64 FMA peak plus the other steps at the "
-                    "measured FP32 FMA peak, divisions and square roots as one flop (FP32 divisions and "
-                    "square roots run on the multi-function unit, whose measured rates are in the line's "
-                    "peaks: fp32_fdividef_gops, fp32_sqrt_gops), op mix per step from "
-                    "the oracle's op-counting build (IS weights in one-division form); frac = roofline "
-                    "time / CUDA-event time of one launch (of measured), from %d steps timed per kernel "
-                    "right after the graph-replayed timed steps" % (MIXED_FP64_STEPS, PROFILE_STEPS_MIXED)}
+            "avg_launch_ms": avg_ms, "traffic": None}
+
+
+def mixed_roofline(ops, peaks, avg_ms, ncell, fallbacks):
+    """Roofline of the dominant mixed sweep: FP64 node, update and combine
+    steps, the others (the wave-speed maximum, reduced in FP32 in the combine
+    epilogue, included) in FP32."""
+    r = two_pipes(ops, peaks, avg_ms, ncell, MIXED_FP64_STEPS)
+    r["fp64_fallbacks"] = fallbacks
+    r["note"] = ("mixed sweep: FP64 steps %s at the measured FP64 FMA peak plus the other steps at the "
+                 "measured FP32 FMA peak, divisions and square roots as one flop (FP32 divisions and "
+                 "square roots run on the multi-function unit, whose measured rates are in the line's "
+                 "peaks: fp32_fdividef_gops, fp32_sqrt_gops), op mix per step from "
+                 "the oracle's op-counting build (IS weights in one-division form); frac = roofline "
+                 "time / CUDA-event time of one launch (of measured), from %d steps timed per kernel "
+                 "right after the graph-replayed timed steps" % (MIXED_FP64_STEPS, PROFILE_STEPS_MIXED))
+    return r
 
 
 def fp64_roofline(ops, peaks, avg_ms, ncell, kernel):
     """Roofline of one launch of an FP64 sweep (one direction over ncell
     cells): the oracle's op mix per cell and direction, every add, mul,
-    min/max, division and square root one flop, over the launch time,
-    against the measured FP64 FMA peak.  frac_div_sqrt_weighted counts each
-    division and square root at its measured cost in FMA-flops instead."""
+    min/max, division and square root one flop, each step on the pipe that
+    it runs on.  frac_fp64_pipe_alone holds all of it against the FP64 FMA
+    peak (above 1 by what does not run there); frac_div_sqrt_weighted is
+    that with each division and square root at its measured cost in
+    FMA-flops."""
+    r = two_pipes(ops, peaks, avg_ms, ncell, FP64_PIPE_STEPS)
     p64 = peaks.get("fp64_fma_tflops", 1.25)
     div_eq = (p64 * 1e12) / (peaks.get("fp64_div_gops", 67.0) * 1e9)
     sqrt_eq = (p64 * 1e12) / (peaks.get("fp64_sqrt_gops", 58.5) * 1e9)
     plain = ops["add"] + ops["mul"] + ops["minmax"] + ops["div"] + ops["sqrt"]
     weighted = ops["add"] + ops["mul"] + ops["minmax"] + div_eq * ops["div"] + sqrt_eq * ops["sqrt"]
-    t = avg_ms * 1e-3
-    achieved = plain * ncell / t / 1e12
-    return {"bound": "alu", "achieved": achieved, "peak": p64, "unit": "TFLOP/s", "frac": achieved / p64,
-            "traffic": None, "kernel": kernel, "avg_launch_ms": avg_ms,
-            "flops_per_cell_dir": plain,
-            "frac_div_sqrt_weighted": weighted * ncell / t / 1e12 / p64,
-            "flop_eq_per_cell_dir_div_sqrt_weighted": weighted,
-            "ops_per_cell_dir": {k: v for k, v in ops.items() if k != "per_step"},
-            "peak_source": peaks.get("source", "nominal FP64 1.25 TFLOP/s (fallback)"),
-            "note": "FP64-pipe roofline of the dominant sweep: algorithmic flops = the oracle's op mix per cell "
-                    "and direction (op-counting build, IS weights in their one-division form), add, mul, "
-                    "min/max, division and square root one flop each, x cells of one launch, over the launch's "
-                    "live CUDA-event time; peak = the FP64 FMA rate of this GPU measured live (of measured). "
-                    "frac_div_sqrt_weighted counts each division / square root at its measured cost in "
-                    "FMA-flops (%.1f / %.1f).  A fraction above 1 means that part of these flops does not run "
-                    "on the FP64 pipe: the sweeps evaluate the IS weights, the HCS combination and the idle "
-                    "limiters' tests on the FP32 and integer pipes to FP64 accuracy" % (div_eq, sqrt_eq)}
+    rate = ncell / (avg_ms * 1e-3) / 1e12 / p64
+    r.update({"kernel": kernel, "flops_per_cell_dir": plain, "frac_fp64_pipe_alone": plain * rate,
+              "frac_div_sqrt_weighted": weighted * rate, "flop_eq_per_cell_dir_div_sqrt_weighted": weighted,
+              "ops_per_cell_dir": {k: v for k, v in ops.items() if k != "per_step"},
+              "peak_source": peaks.get("source", "nominal FP64 1.25 TFLOP/s (fallback)"),
+              "note": "dominant FP64 sweep: steps %s at the measured FP64 FMA peak plus the others (IS weights, HCS "
+                      "combination, idle limiters' tests, evaluated on the FP32 and integer pipes to FP64 accuracy) at "
+                      "the measured FP32 FMA peak, op mix per step from the oracle's op-counting build (IS weights in "
+                      "one-division form), add, mul, min/max, division and square root one flop each; frac = roofline "
+                      "time / CUDA-event time of one launch (of measured).  frac_fp64_pipe_alone holds every flop "
+                      "against the FP64 pipe; frac_div_sqrt_weighted that with each division / square root at its "
+                      "measured cost in FMA-flops (%.1f / %.1f)" % (FP64_PIPE_STEPS, div_eq, sqrt_eq)})
+    return r
 
 
 # ---------------------------------------------------------------------------
@@ -706,10 +721,9 @@ def algorithmic_ops_1d(rb=None):
 def batch_roofline(ops, peaks, prec, ms_per_step, cells, ndim=1):
     """Step-level roofline fraction of the batched mode: the algorithmic
     work of three RHS evaluations over all cells and directions (every add,
-    mul, min/max, division and square root one flop) at the FP64 pipe's
-    measured rate (FP64) or at the two pipes' rates (mixed, as
-    mixed_roofline), over the whole step's time (the per-problem dt kernel
-    included)."""
+    mul, min/max, division and square root one flop) at the two pipes'
+    measured rates (as fp64_roofline and mixed_roofline), over the whole
+    step's time (the per-problem dt kernel included)."""
     sweeps = 3 * ndim
     if prec == "mixed":
         r = mixed_roofline(ops, peaks, ms_per_step / sweeps, cells, fallbacks=None)
