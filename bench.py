@@ -417,6 +417,18 @@ def dominant(prof, ndim):
     return d, prof["ms"][d] / prof["launches"][d]
 
 
+# Every source of the FP64 sweeps' code (the counters below belong to them).
+KERNEL_SOURCES = ("wcns_sweep.cuh", "wcns_isw.cuh", "wcns_math64.cuh", "wcns_internal.h", "wcns_fp64.cu")
+
+
+def kernel_source_hash():
+    h = hashlib.sha256()
+    for name in KERNEL_SOURCES:
+        with open(os.path.join(ROOT, "paper_2102_05287_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
 def all_sweeps(roof, prof, ndim):
     """Adds the fraction over every sweep launch of the profiled steps (the
     sum of their roofline times over the sum of their CUDA-event times),
@@ -533,8 +545,7 @@ def run_gb300(args, world, rank, local):
     dom, avg_ms = dominant(prof64, 2)
     roofline = all_sweeps(fp64_roofline(ops, peaks, avg_ms, ncell,
                                         "sweep_kernel<2,%d,double> (%s sweep)" % (dom, "xy"[dom])), prof64, 2)
-    src_hash = hashlib.sha256(open(os.path.join(ROOT, "paper_2102_05287_gb300", "csrc", "wcns_sweep.cuh"),
-                                   "rb").read()).hexdigest()[:16]
+    src_hash = kernel_source_hash()
     traffic_file = os.path.join(ROOT, "profiles", "sweep_traffic.json")
     if os.path.exists(traffic_file):
         try:

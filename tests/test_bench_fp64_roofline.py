@@ -1,9 +1,16 @@
-"""bench.py's FP64 roofline (CPU): every step of the
+"""bench.py's FP64 roofline and traffic record (CPU): every step of the
 algorithm is held against the pipe that the FP64 sweeps run it on, so that the
-fraction is one of what bounds the kernel."""
+fraction is one of what bounds the kernel; and the traffic counters are taken
+as a kernel's own only for the sources that make up its code."""
+import os
+import re
+
 import pytest
 
 import bench
+from tests.conftest import ROOT
+
+CSRC = os.path.join(ROOT, "paper_2102_05287_gb300", "csrc")
 
 
 def test_fraction_is_of_both_pipes():
@@ -20,3 +27,32 @@ def test_fraction_is_of_both_pipes():
     assert r["frac"] == pytest.approx(t / (ms * 1e-3)) and r["frac"] < 1
     assert r["achieved"] / r["peak"] == pytest.approx(r["frac"])
     assert r["frac_fp64_pipe_alone"] == pytest.approx(sum(flops.values()) * ncell / 1.25e12 / (ms * 1e-3))
+
+
+def includes(name, seen=None):
+    seen = set() if seen is None else seen
+    if name not in seen and os.path.exists(os.path.join(CSRC, name)):
+        seen.add(name)
+        for inc in re.findall(r'#include "([^"]+)"', open(os.path.join(CSRC, name)).read()):
+            includes(os.path.normpath(inc), seen)
+    return seen
+
+
+def test_traffic_hash_covers_every_source_of_the_sweeps():
+    own = {n for n in includes("wcns_fp64.cu") if not n.startswith("..")}
+    assert set(bench.KERNEL_SOURCES) == own
+
+
+def test_traffic_hash_follows_each_source(monkeypatch, tmp_path):
+    d = tmp_path / "paper_2102_05287_gb300" / "csrc"
+    d.mkdir(parents=True)
+    for n in bench.KERNEL_SOURCES:
+        (d / n).write_bytes(open(os.path.join(CSRC, n), "rb").read())
+    h = bench.kernel_source_hash()
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    assert bench.kernel_source_hash() == h
+    for n in bench.KERNEL_SOURCES:
+        text = (d / n).read_bytes()
+        (d / n).write_bytes(text + b"\n")
+        assert bench.kernel_source_hash() != h, n
+        (d / n).write_bytes(text)
