@@ -72,9 +72,9 @@ struct BatchGeo {
 // MIXED selects the mixed-precision body (wcns_mixed_body.cuh).  Mixed
 // tiles target BATCH_MIXED_WARPS resident warps per SM (a register cap of
 // 65536 / (32 BATCH_MIXED_WARPS) per thread), FP64 tiles BATCH_FP64_WARPS
-// (4096 problems: 8 / 12 / 16 / 20 warps 23.3 / 21.6 / 21.5 / 21.9 ms a
-// step).  On the 4096-problem batch 32 warps (64 registers, more
-// spills) beat 28, 24, 20 and 16: the single-pass body is latency bound.
+// (4096 problems: 12 / 16 / 20 warps 16.1 / 16.2 / 16.7 ms a step).  On the
+// 4096-problem batch 32 warps (64 registers, more spills) beat 28, 24, 20 and
+// 16 for mixed tiles: the single-pass body is latency bound.
 #ifndef BATCH_FP64_WARPS
 #define BATCH_FP64_WARPS 16
 #endif

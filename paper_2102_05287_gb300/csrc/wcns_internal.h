@@ -128,9 +128,9 @@ inline int status_from_counts(const StepCtl &c, const DevStats &s, int ok, int e
 // that nothing writes during the kernel's life, and that life begins before
 // the wait.  Only for grids whose blocks are all resident with room to
 // spare: waiting blocks of a large grid would hold the predecessor's slots.
-// One step of a 200-cell FP64 shock tube 124 -> 119.5 us, ten of a 512-cell run
-// 551 -> 530 us.
-constexpr long long EARLY_MAX_BLOCKS = 304;
+// One step of a 200-cell FP64 shock tube 124 -> 119 us, ten of a 512-cell run
+// 544 -> 536 us, a 136 x 136 step (272 blocks a sweep) 458 -> 443 us.
+constexpr long long EARLY_MAX_BLOCKS = 2 * 152;  // two blocks on each of GB300's 152 SMs
 __device__ __forceinline__ void after_predecessor() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
